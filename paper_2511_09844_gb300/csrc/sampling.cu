@@ -236,6 +236,7 @@ __global__ void __launch_bounds__(kRowThreads) row_stats_kernel(const T* target,
                                                                 const float* temp, const int* stopped,
                                                                 AcceptScratch sc, unsigned* err, int reset_err) {
   pdl_trigger();
+  cluster_arrive_relaxed();                          // waited for before the first store into another CTA
   pdl_wait();
   __shared__ unsigned long long red[32];
   __shared__ __align__(16) float4 sMax[C];           // from every CTA: key (two words), non-finite flag
@@ -253,6 +254,10 @@ __global__ void __launch_bounds__(kRowThreads) row_stats_kernel(const T* target,
       const int v = lo + (u * kRowThreads + static_cast<int>(threadIdx.x)) * 8;
       load8<T>(row, v, max(0, hi - v), z[u]);
     }
+  // Every CTA of the cluster runs: a store into the shared memory of one that has not started would be lost (a
+  // short vocabulary leaves slices empty, whose CTAs are at their stores at once). The row's loads are under way.
+  __syncwarp();
+  cluster_wait();
   if (rank == 0) prepare_race(r, B, k, sc, err, reset_err);
   if (stopped && stopped[rr.b]) return;              // uniform over the cluster
   const float t = temp[rr.b];

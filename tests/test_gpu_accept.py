@@ -188,3 +188,19 @@ def test_zero_residual_falls_back_to_the_target_row():
         draft[:, :, 3] = -67.0
         js = _compare(target, draft, torch.full((B, k), 3, dtype=torch.int32), [1.0] * B, seed=5, step=1)
         assert js == [0] * B
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V,B,k", [(4, 1, 1), (8, 2, 2), (36, 1, 5), (132, 3, 4), (516, 5, 3), (1020, 9, 4)])
+def test_vocabularies_shorter_than_a_cluster_s_slices(dtype, V, B, k):
+    """Few rows of so short a vocabulary that CTAs of a row's cluster have no entries and are at once where they
+    exchange their maxima; many blocks in a row, so that clusters start at all times."""
+    target, draft, xhat = W.make_sweep_logits(B, k, V, seed=V + B + k, share_prob=0.8)
+    temps = [[1.0, 0.0, 0.7][b % 3] for b in range(B)]
+    tt = torch.tensor(temps, dtype=torch.float32, device="cuda")
+    t, d, x = target.to(dtype).cuda(), draft.to(dtype).cuda(), xhat.cuda()
+    got = [sd2.accept_logits(t, d, x, tt, 7, step) for step in range(40)]
+    torch.cuda.synchronize()
+    for step, (tok, n) in enumerate(got):
+        for b, (emitted, j) in enumerate(_oracle(t, d, xhat, temps, 7, step)):
+            assert int(n[b]) == j + 1 and tok[b, :j + 1].tolist() == emitted, (step, b)
