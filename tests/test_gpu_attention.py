@@ -371,3 +371,29 @@ def test_few_query_vectors_over_many_sequences(H, Hkv, k1, n_seq, stable_off):
         out, err = _run_flat(c, n_seq, max(lens) + 16, kw["pre_len"], -1, kw["pre_fresh"])
         assert err == 0
         _check(out, ref)
+
+
+@pytest.mark.parametrize("kind,hd,H,Hkv,k1", [("prompt", 128, 8, 2, 0), ("prompt", 64, 14, 2, 0), ("splits", 128, 32, 8, 1),
+                                              ("splits", 128, 16, 4, 6), ("splits", 128, 8, 2, 16), ("splits", 64, 8, 2, 4),
+                                              ("flat", 128, 8, 2, 9), ("flat", 64, 8, 2, 9)])
+def test_probabilities_enter_the_products_unrounded(kind, hd, H, Hkv, k1):
+    """The tcgen05 kernels form probabilities about a reference below the row's maximum, so even the largest is
+    not exactly 1: they enter P V in two bf16 parts. What is left of the error against 64 bits on the same bf16
+    queries, keys and values is the rounding of the result (2^-9 at most; the parts leave 2^-17, sums in f32 less):
+    one bf16 part alone adds as much again, 1.2 to 1.4 times the rounding's error in all."""
+    if kind == "prompt":
+        c = _prompt_case(25, [900], [0], H, Hkv, hd)
+        ref = _prompt_reference(c)
+        out, err = _run(c, 1, 960, max_rows=64 // (H // Hkv))
+    elif kind == "splits":
+        c = _case(26, [4096], [k1], H, Hkv, hd)
+        ref = _reference(c)
+        out, err = _run(c, 16, 256)
+    else:
+        lens = [k1 + (311 * i) % (64 * 24) for i in range(13)]
+        c = _case(27, lens, [k1] * 13, H, Hkv, hd)
+        ref = _reference(c)
+        out, err = _run_flat(c, 36, 64 * 24 + 64, [L - k1 + 1 for L in lens], -1, k1 + 1)
+    assert err == 0
+    rounding = (ref.to(torch.bfloat16).double() - ref).norm()
+    assert (out.double() - ref).norm() <= 1.05 * rounding
