@@ -255,7 +255,8 @@ __global__ void swiglu_kernel(const float* gate, const float* up, const float* b
   }
 }
 
-// blockIdx.y = row, blockIdx.x = slice of kGatherSpan entries: 8 consecutive ones a thread, so a row of
+// blockIdx.x = row (a batch may exceed the 65535 of the other grid dimensions), blockIdx.y = slice of kGatherSpan
+// entries: 8 consecutive ones a thread, so a row of
 // 12288 is 6 CTAs of one load round (one CTA walking it entry by entry took 24 us, cold).
 constexpr int kGatherSpan = 256 * 8;
 __global__ void __launch_bounds__(256) gather_rows_bf16_kernel(const float* __restrict__ src, int ld_src,
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(256) gather_rows_bf16_kernel(const float* __re
                                                                bf16* __restrict__ out) {
   pdl_trigger();
   pdl_wait();
-  const int b = blockIdx.y, j = blockIdx.x * kGatherSpan + threadIdx.x * 8;
+  const int b = blockIdx.x, j = blockIdx.y * kGatherSpan + threadIdx.x * 8;
   if (j >= width) return;
   const float* s = src + static_cast<size_t>(b) * ld_src + static_cast<size_t>(idx ? idx[b] : 0) * width + j;
   bf16* o = out + static_cast<size_t>(b) * width + j;
@@ -336,7 +337,7 @@ cudaError_t swiglu(const float* gate, const float* up, const float* bias, const 
 cudaError_t gather_rows_bf16(const float* src, int ld_src, const int* idx, int width, int B, void* out,
                              cudaStream_t st) {
   if (B <= 0 || width <= 0) return cudaSuccess;
-  { const cudaError_t e_ = launch_pdl(gather_rows_bf16_kernel, dim3((width + kGatherSpan - 1) / kGatherSpan, B), dim3(256), 0, st, src, ld_src, idx, width, static_cast<bf16*>(out)); if (e_ != cudaSuccess) return e_; }
+  { const cudaError_t e_ = launch_pdl(gather_rows_bf16_kernel, dim3(B, (width + kGatherSpan - 1) / kGatherSpan), dim3(256), 0, st, src, ld_src, idx, width, static_cast<bf16*>(out)); if (e_ != cudaSuccess) return e_; }
   return cudaGetLastError();
 }
 

@@ -330,3 +330,18 @@ def test_prompt_projections_on_cta_pairs(heads, kv_heads, hd, lens):
     prompts = W.make_prompts(work.verifier.vocab, 3, lens, seed=42)
     rep = parity.run(work, vw, dw, st, prompts, [0.0, 0.7, 1.0], seed=43, n_steps=2)
     assert rep.blocks == 6
+
+
+@pytest.mark.parametrize("B", [1, 3, 65535, 65536, 70001])
+def test_standalone_steering_of_any_batch(B):
+    """sd2_steer against 64 bits on the same bf16 taps, also with more sequences than a grid's y dimension holds."""
+    dv, dg, nb = 64, 128, 128
+    g = torch.Generator(device="cuda").manual_seed(B)
+    bf = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    st = {"w_hml": bf(dg, 3 * dv), "w_s": bf(nb, dg), "ln_gamma": bf(dg), "ln_beta": bf(dg)}
+    taps = torch.randn(B, 3, dv, generator=g, device="cuda")
+    out, bias = sd2.steer(taps, st, 1e-5, nb)
+    x = taps.to(torch.bfloat16).double().reshape(B, -1) @ st["w_hml"].double().T
+    ref = torch.nn.functional.layer_norm(x, (dg,), st["ln_gamma"].double(), st["ln_beta"].double(), 1e-5)
+    torch.testing.assert_close(out.double(), ref, atol=2e-5, rtol=2e-5)              # f32 sums of 192 and 128 terms
+    torch.testing.assert_close(bias.double(), out.to(torch.bfloat16).double() @ st["w_s"].double().T, atol=2e-4, rtol=2e-5)
