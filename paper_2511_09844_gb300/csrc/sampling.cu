@@ -921,9 +921,10 @@ __global__ void __launch_bounds__(kThreads) sample_kernel(const float* logits, l
     }
   }
   best = block_max_u64(best, red);
+  const int any_bad = __syncthreads_or(bad ? 1 : 0);
   if (threadIdx.x == 0) {
     atomicMax(&slot[b], best);
-    if (bad) atomicOr(err, static_cast<unsigned>(ERR_NONFINITE));
+    if (any_bad) atomicOr(err, static_cast<unsigned>(ERR_NONFINITE));
     __threadfence();
     last = (atomicAdd(&counter[b], 1) == static_cast<int>(gridDim.y) - 1);
   }

@@ -2,6 +2,8 @@
 
 * an allocation failure injected at several points of sd2_init returns SD2_ENOMEM and leaves no
   device memory behind; a context made afterwards works;
+* a non-finite logit at any place of a sampled row (the first token's, a draft's) is reported, and the
+  context goes on;
 * a bounded device wait that nothing satisfies, with a short budget set by the test, gives up,
   latches the time-out and returns: sd2_check reports SD2_ETIMEOUT, and the context goes on to
   produce exactly the tokens of a context that never saw it.
@@ -75,3 +77,24 @@ def test_bounded_wait_expiry_is_reported_and_the_context_stays_usable():
         runs.append(_tokens(eng, 4, probe))
         eng.close()
     assert runs[0] == runs[1]
+
+
+@pytest.mark.parametrize("which,place", [("verifier", 0), ("verifier", 1), ("verifier", 517), ("verifier", -1), ("drafter", 2),
+                                         ("drafter", 1000), ("drafter", -1)])
+def test_nonfinite_logits_of_sampled_rows_are_reported(which, place):
+    """A NaN in one row of the head makes that entry of every logit row NaN: thread 0 of a sampling block sees
+    entries 0 .. 3 of every 1024, the others belong to other threads. The first token's row is read by the
+    sampling kernel alone, and so are the draft rows of a greedy sequence."""
+    work = parity.tiny_work()
+    dev_w = [parity.to_device(w) for w in parity.tiny_weights(work)]
+    dev_w[0 if which == "verifier" else 1]["lm_head"][place, 0] = float("nan")
+    eng = _engine(work, dev_w)
+    eng.prefill(W.make_prompts(work.verifier.vocab, 2, (20, 30), seed=3), [0.0, 0.0], seed=5)
+    if which == "drafter":
+        eng.check()                       # the prompt samples no drafter row
+        eng.step()
+    with pytest.raises(sd2.SD2Error) as e:
+        eng.check()
+    assert e.value.status == sd2.SD2_ENUMERIC
+    eng.check()                           # the word was cleared
+    eng.close()
