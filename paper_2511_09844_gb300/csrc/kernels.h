@@ -312,6 +312,8 @@ struct AcceptScratch {
   unsigned long long minus_zero2;   // kMinusZero2 (common.cuh)
 };
 size_t accept_scratch_bytes(int B, int k);
+// Bound on the relative error of a row's approximate softmax normaliser (the path of many rows).
+float accept_norm_margin(int V);
 // Philox key of the sampling kernels: `value`, or the word at `ptr` when ptr is set (so that a
 // captured step can take a new request's seed without being captured again).
 struct Seed {

@@ -338,12 +338,15 @@ __global__ void __launch_bounds__(kRowThreads) row_stats_kernel(const T* target,
 // instead of on all 2k + 1 of a sequence. What is left per logit, about 6 operations and one ex2,
 // fits under the one read of the logits: 256 sequences x 33 rows of 152064 bf16 take 462 us in all for
 // 2.57 GB (5.6 TB/s), 1928 us with two passes and the exact exponential of every logit.
-// Relative error of the approximate normaliser against the exact one (norm_margin): the exponents'
-// roundings (two subtractions and a product at |t| <= 32: 4e-6; smaller e contribute less than
-// V 2^-45 in all), ex2 and exp_cw themselves (4e-7), the fp32 sums (a thread's chain of
-// V / (4 threads) per accumulator, and the block's tree).
+// Relative error of the approximate normaliser against the exact one (accept_norm_margin), with u = 2^-24:
+//   exponents    three roundings of the distance t from the maximum (the exact side's subtraction; a subtraction,
+//                and the product with a rounded log2 e, here; a chain of references splits t, not the errors'
+//                sum), weighted by the mass at t, whose mean is at most ln V: 13 (3 u + 2^-26) < 3e-6
+//   ex2, exp_cw  4e-7
+//   sums         u for every entry of a thread's accumulator (V / (4 threads)) and for the block's tree
+//   rescales     ex2 (2^-22) and a product (u) for every raise of a thread's reference, at most one a pass of 32
+//                entries a thread, one for the last 4 entries and one to the block's maximum
 constexpr int kManyThreads = 256;
-float norm_margin(int V) { return 6e-6f + 6.0e-8f * (static_cast<float>(V) / (4.f * kManyThreads) + 24.f); }
 
 constexpr float kLog2e = 0x1.715476p+0f;
 
@@ -995,7 +998,7 @@ cudaError_t accept_typed(const T* target, const T* draft, const int* xhat, const
   e = launch_pdl(row_scan_kernel<T>, dim3(R), dim3(kManyThreads), 0, st, target, draft, B, k, V, temp, stopped, s, err, reset);
   if (e != cudaSuccess) return e;
   // p and u q each carry one normaliser's error; a few fp32 roundings on top
-  const float margin = 2.f * norm_margin(V) + 1e-6f;
+  const float margin = 2.f * accept_norm_margin(V) + 1e-6f;
   e = launch_pdl(decide_kernel<T>, dim3(B), dim3(kRowThreads), 0, st, target, draft, xhat, temp, B, k, V, seed, step_ptr,
                  step, stopped, tokens, n, s, err, margin);
   if (e != cudaSuccess) return e;
@@ -1007,6 +1010,11 @@ cudaError_t accept_typed(const T* target, const T* draft, const int* xhat, const
 }
 
 }  // namespace
+
+float accept_norm_margin(int V) {
+  const int passes = (V + 32 * kManyThreads - 1) / (32 * kManyThreads);
+  return 6e-6f + 6.0e-8f * (static_cast<float>(V) / (4.f * kManyThreads) + 24.f) + 3.1e-7f * static_cast<float>(passes + 2);
+}
 
 size_t accept_scratch_bytes(int B, int k) {
   const size_t R = static_cast<size_t>(B) * (2 * k + 1);

@@ -1,6 +1,7 @@
 """Host-side checks of the C ABI (no GPU): the library builds, loads and exports every function
 include/sd2.h declares, and the Python mirrors of its structs have the C layout."""
 import ctypes
+import math
 import os
 import re
 import subprocess
@@ -135,3 +136,18 @@ def test_standalone_entry_points_check_arguments_on_the_host(lib):
     assert err_is(flat(n_groups=65, slots=100), b"flat mode")
     assert err_is(flat(n_groups=3, slots=2), b"flat mode")
     assert err_is(flat(max_ctx=64), b"flat mode")
+
+
+def test_margin_of_the_approximate_normaliser_covers_its_error_terms(lib):
+    """Acceptance of many rows decides from a normaliser summed by the hardware's ex2 in f32 about a running
+    reference, wherever that cannot change a decision: its margin must be no less than the sum of its error terms,
+    the rescales at every raise of the reference (one a pass of 32 entries of 256 threads at most) among them."""
+    margin = lib._ZN3sd218accept_norm_marginEi
+    margin.restype, margin.argtypes = ctypes.c_float, [ctypes.c_int]
+    u, ex2 = 2.0 ** -24, 2.0 ** -22                     # an f32 rounding; ex2.approx, by its documentation
+    for V in [4, 1000, 8192, 8196, 32000, 65536, 128256, 152064, 256000, 400000]:
+        exponents = max(1.0, math.log(V)) * (3 * u + 2.0 ** -26)
+        sums = (V / 1024 + 24) * u
+        rescales = (-(-V // 8192) + 1) * (ex2 + u)
+        total = exponents + 4e-7 + sums + rescales
+        assert total <= margin(V) < 2 * total + 1e-5, (V, total, margin(V))

@@ -204,3 +204,23 @@ def test_vocabularies_shorter_than_a_cluster_s_slices(dtype, V, B, k):
     for step, (tok, n) in enumerate(got):
         for b, (emitted, j) in enumerate(_oracle(t, d, xhat, temps, 7, step)):
             assert int(n[b]) == j + 1 and tok[b, :j + 1].tolist() == emitted, (step, b)
+
+
+def test_close_calls_on_rows_whose_maximum_keeps_rising():
+    """The largest vocabulary, logits that rise along it, so that every thread raises its reference in every pass;
+    u q and p within a few ulps of each other."""
+    from oracle import philox
+    B, k, V, seed, step = 52, 1, 152064, 33, 4
+    g = torch.Generator().manual_seed(12)
+    rise = torch.linspace(0, 9, V, dtype=torch.float64)
+    draft = torch.randn(B, k, V, generator=g, dtype=torch.float64) * 0.05 + rise
+    target = torch.randn(B, k + 1, V, generator=g, dtype=torch.float64) * 0.05 + rise
+    xhat = torch.randint(0, V, (B, k), generator=g, dtype=torch.int32)
+    for b in range(B):
+        x, u = int(xhat[b, 0]), float(philox.accept_uniform(seed, 1, b, step))
+        q = float(torch.softmax(draft[b, 0], 0)[x])
+        want = u * q * (1 + 2e-7 * float(torch.randn(1, generator=g)))
+        rest = torch.cat([target[b, 0, :x], target[b, 0, x + 1:]]).logsumexp(0)
+        target[b, 0, x] = float(rest) + np.log(want / (1 - want))            # p(x) = want
+    js = _compare(target.float(), draft.float(), xhat, [1.0] * B, seed, step)
+    assert set(js) == {0, 1}
