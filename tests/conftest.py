@@ -23,3 +23,19 @@ def golden_rows(name):
             if line:
                 rows.append(line.split())
     return rows
+
+
+def kernels_of(fn):
+    """Names of the kernels that fn() launches (graph launches included), as the profiler sees them. A process's
+    first profile may come back empty: fn() is run again then."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(3):
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as p:
+            fn()
+            torch.cuda.synchronize()
+        names = {e.name for e in p.events() if "kernel" in e.name}
+        if names:
+            break
+    return names

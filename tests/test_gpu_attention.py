@@ -14,6 +14,7 @@ word, not fault.
 import pytest
 import torch
 
+from conftest import kernels_of
 from oracle import model as oracle_model
 from paper_2511_09844_gb300 import sd2
 
@@ -266,13 +267,15 @@ def _prompt_reference(c):
 @pytest.mark.parametrize("hd,H,Hkv", [(128, 32, 8), (64, 32, 8), (64, 14, 2), (128, 4, 4), (64, 64, 1)])
 @pytest.mark.parametrize("lens,first", [([300], [0]), ([64], [0]), ([17, 130, 1], [0, 0, 0]), ([200, 450], [150, 33])])
 def test_prompt_rows(hd, H, Hkv, lens, first):
-    """Whole prompts and the later rows of prompts (the tcgen05 kernel): pairs of groups within one
+    """Whole prompts and the later rows of prompts (the tcgen05 kernel, which takes launches of eight tiles): pairs of groups within one
     sequence and across two, an odd number of groups, groups of 64, 63 and fewer query vectors, tiles
     partly past the prompt's end whose cache rows are not finite."""
     c = _prompt_case(12, lens, first, H, Hkv, hd)
-    out, err = _run(c, 1, 64 * ((max(lens) + 63) // 64), max_rows=64 // (H // Hkv))
-    assert err == 0
-    _check(out, _prompt_reference(c))
+    ref = _prompt_reference(c)
+    for chunk in (64 * ((max(lens) + 63) // 64), 64 * 8):      # by its length a short prompt runs on the general kernel
+        out, err = _run(c, 1, chunk, max_rows=64 // (H // Hkv))
+        assert err == 0
+        _check(out, ref)
 
 
 def test_prompt_scores_that_keep_rising():
@@ -345,9 +348,27 @@ def test_prompt_rows_four_groups_a_cta(hd, H, Hkv, lens, first):
     """CTAs whose four groups lie in one, two and more sequences (a pass each), halves of unequal contexts and
     empty ones, contexts that end in a partial cache block, on a tile's edge and one row past it."""
     c = _prompt_case(23, lens, first, H, Hkv, hd)
-    out, err = _run(c, 1, 64 * ((max(lens) + 63) // 64), max_rows=64 // (H // Hkv))
+    out, err = _run(c, 1, max(64 * 8, 64 * ((max(lens) + 63) // 64)), max_rows=64 // (H // Hkv))
     assert err == 0
     _check(out, _prompt_reference(c))
+
+
+def _kernel(c, *args, **kw):
+    """The attention kernel a launch of c runs on."""
+    names = [n for n in kernels_of(lambda: _run(c, *args, **kw)) if "attn" in n]
+    assert len(names) == 1, names
+    return next(k for k in ("attn_prompt", "attn_few", "attn_stream", "attn") if k + "_kernel" in names[0])
+
+
+@pytest.mark.parametrize("hd,H,Hkv,lens,kernel", [
+    (128, 32, 8, [17], "attn"), (128, 32, 8, [64, 27, 1, 1], "attn"), (128, 32, 8, [256], "attn"),
+    (128, 32, 8, [192, 155, 118, 81], "attn_prompt"), (128, 32, 8, [321], "attn_prompt"), (128, 8, 2, [300], "attn"),
+    (64, 32, 8, [256], "attn_prompt"),
+    (64, 14, 2, [192, 155, 118, 81], "attn"), (64, 14, 2, [256, 219, 182, 145], "attn_prompt"), (64, 14, 2, [384], "attn_prompt")])
+def test_short_prompts_run_on_the_general_kernel(hd, H, Hkv, lens, kernel):
+    """Prompts of a few tiles and few CTAs are quicker on many small CTAs than on the tcgen05 kernel's."""
+    c = _prompt_case(28, lens, [0] * len(lens), H, Hkv, hd)
+    assert _kernel(c, 1, 64 * ((max(lens) + 63) // 64), max_rows=64 // (H // Hkv)) == kernel
 
 
 @pytest.mark.parametrize("H,Hkv,k1,n_seq", [(32, 8, 1, 8), (32, 8, 4, 9), (14, 2, 1, 32), (14, 2, 2, 40), (16, 16, 9, 8), (32, 8, 2, 30)])
