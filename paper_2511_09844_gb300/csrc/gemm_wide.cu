@@ -18,6 +18,7 @@
 // 394 -> 252 us (1.86 PFLOP/s; cuBLAS reaches 1.98 on 8192^3), 8000 rows 1507 -> 989; 8000 rows
 // x 14336 -> 4096 1009 -> 522; x 4096 -> 6144 280 -> 235. Prefill of 8352 prompt tokens through the
 // 8B/1B pair 206 -> 100 ms, of 512 25.6 -> 9.7.
+// Between 129 and 192 rows short and very long weight matrices stay there (weights_as_m_rows).
 //
 // Work split. Tiles are walked in groups of kGroupTiles token tiles, weight tiles slowest, so a
 // group's tokens stay in L2 while the weights pass once per group. With fewer tiles than resident
@@ -48,7 +49,6 @@ constexpr int kEpiWarps = 8;                  // two per TMEM lane quarter, taki
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kUnits = 8;                     // units of 32 accumulator columns in a tile
 constexpr int kMaxSplit = 4;
-constexpr int kWideMinSplitRows = 144;
 constexpr int kGroupTiles = 8;                // token tiles walked together
 constexpr int kPatchBytes = 32 * 32 * 4;       // a warp's transposing patch of the f32 epilogues
 constexpr int kSmem = 1024 + kStages * kStageBytes + kEpiWarps * kPatchBytes + 512;
@@ -666,6 +666,35 @@ cudaError_t launch_wide(const WideArgs& a, const WidePlan& pl, cudaStream_t st) 
 
 }  // namespace
 
+// Rows up to which the weights-as-M kernel keeps a launch. Against a short weight matrix this kernel's few tiles split
+// K four ways on at most 136 SMs, where the other one spreads the same weights over more CTAs; a very long one is a
+// weight stream of several waves either way, which the other one starts sooner. Both, us (here / there), weights cold:
+//   rows                             144            160            168            192
+//     896 x 4864, residual add   14.5 / 11.1    14.5 / 12.3    14.5 / 12.9    14.5 / 13.2    (200: 14.5 / 15.9)
+//    1024 x 1024, residual add   10.0 / 9.1     10.1 / 9.7     10.1 / 10.4    10.1 / 10.5
+//    2048 x 8192, residual add   19.5 / 16.7    19.5 / 18.6    19.5 / 19.5    19.5 / 24.8
+//    2816 x 12800, residual add  25.6 / 22.1    25.6 / 24.6
+//    3328 x 12800, residual add  26.0 / 24.0    26.1 / 28.2
+//    3840 x 6400, residual add   19.6 / 18.3    19.7 / 20.6
+//    4096 x 4096, residual add   17.7 / 15.3    17.6 / 17.0    17.7 / 18.1    17.7 / 18.1
+//    4096 x 14336, residual add  33.0 / 29.1    33.1 / 33.1    33.1 / 34.3    33.1 / 34.7
+//    4608 x 6400, residual add   21.7 / 19.0    21.7 / 21.3
+//    4864 x 6400, residual add   21.9 / 22.3    22.0 / 24.9
+//    5120 x 27648, residual add  56.3 / 60.0    56.4 / 68.7    56.3 / 70.3    56.6 / 105
+//   32768 x 2048, stored         28.7 / 28.6    28.8 / 29.2    28.8 / 29.8    28.9 / 30.2
+//   49152 x 2048, stored         40.3 / 38.4    40.1 / 39.3    40.0 / 39.8    40.7 / 41.1
+//  128256 x 2048, stored         99.6 / 96.2   102.2 / 98.6   103.3 / 103.4  105.5 / 106.3
+//  151936 x 896, stored          65.1 / 58.3    64.6 / 60.5    65.4 / 63.0    67.3 / 65.8
+//   SwiGLU: 1024 x 4096          14.4 / 14.4    14.4 / 15.5;  2048 x 2048 13.7 / 14.1;  14336 x 4096 50.3 / 61.3
+// (The other kernel's K splits fit the SMs worst from 3072 to 4095 features: 24 to 31 tiles.)
+int weights_as_m_rows(const GemmArgs& g) {
+  const int N = out_features(g);
+  if (g.epi == EPI_SWIGLU) return N <= 1024 ? 144 : 0;
+  if (N < 1024) return 192;
+  if (N < 3072 || (N >= 4096 && N <= 4608) || N > 40960) return 160;
+  return N < 4096 ? 144 : 0;
+}
+
 // Whether gemm_tc runs these arguments (already accepted by gemm_tc_supported) on this kernel.
 bool gemm_wide_takes(const GemmArgs& g) {
   if (g.M < kWideMinRows || g.attn_q) return false;
@@ -679,12 +708,7 @@ bool gemm_wide_takes(const GemmArgs& g) {
   }
   if (g.epi != EPI_STORE && g.epi != EPI_QKV && g.bias && (!al16(g.bias) || g.ld_bias % 4)) return false;
   if (g.norm_out && (!al16(g.norm_out) || !al16(g.norm_gamma) || g.ldo % 8 || (g.tap_mask && !al16(g.tap)))) return false;
-  const WidePlan pl = plan_wide(g);
-  // A few hundred rows against a short weight matrix split K three ways or more here, on at most 96 to
-  // 120 SMs; up to 144 rows the weights-as-M kernel spreads the same weights over more CTAs
-  // (144 rows, 14336 -> 4096: 31.1 us there, 33.2 here; 8192 -> 2048: 19.2 and 20.8). At 200 rows it
-  // is this kernel's again (34.5 us against 52.8).
-  return pl.sp > 0 && !(g.M <= kWideMinSplitRows && pl.sp >= 3);
+  return g.M > weights_as_m_rows(g) && plan_wide(g).sp > 0;
 }
 
 int gemm_wide_norm_parts(const GemmArgs& g) {

@@ -4,6 +4,7 @@ import pytest
 import torch
 
 import parity
+from conftest import kernels_of
 from oracle import model as omodel
 from paper_2511_09844_gb300 import sd2
 
@@ -116,7 +117,8 @@ def test_implementations_agree_and_repeat():
 # outside the matrix, K split over 1 to 4 pairs, one k-block (a single accumulator), several tiles per
 # pair, and launches below its row bound or without 16-byte alignment (the other kernel).
 WIDE = [(129, 128, 64), (256, 384, 128), (257, 896, 896), (255, 4096, 1024), (385, 4096, 2048), (150, 2048, 8192),
-        (1025, 2432, 320), (2048, 4096, 192), (144, 4096, 4096), (128, 1152, 896)]
+        (1025, 2432, 320), (2048, 4096, 192), (144, 4096, 4096), (128, 1152, 896), (129, 5120, 64), (193, 128, 64),
+        (192, 896, 128), (161, 2048, 8192), (160, 4352, 128), (145, 3200, 256), (129, 41088, 64), (161, 41088, 64)]
 
 
 @pytest.mark.parametrize("M,N,K", WIDE)
@@ -184,3 +186,17 @@ def test_store_of_several_owner_passes(M, N, K):
     y = sd2.gemm(x.cuda(), w.cuda(), epilogue=0, impl=2)
     torch.cuda.synchronize()
     assert parity.row_rel_err(y, x.float() @ w.float().T) < TOL
+
+
+@pytest.mark.parametrize("M,N,K,epi,wide", [
+    (144, 4096, 4096, 1, False), (160, 2048, 8192, 0, False), (161, 2048, 8192, 1, True), (144, 5120, 2048, 1, True),
+    (192, 896, 1024, 1, False), (193, 896, 1024, 1, True), (160, 2944, 2048, 0, False), (144, 3840, 2048, 0, False), (145, 3840, 2048, 0, True),
+    (144, 49152, 1024, 0, False), (161, 49152, 1024, 0, True), (144, 8192, 2048, 2, True), (144, 1024, 2048, 2, False),
+    (128, 8192, 2048, 2, False)])
+def test_which_kernel_takes_a_hundred_and_more_rows(M, N, K, epi, wide):
+    """Either side of every line between the weights-as-M kernel and the CTA-pair kernel."""
+    x, w = torch.zeros(M, K, dtype=torch.bfloat16, device="cuda"), torch.zeros(N, K, dtype=torch.bfloat16, device="cuda")
+    out = torch.zeros(M, N, device="cuda")
+    names = kernels_of(lambda: sd2.gemm(x, w, epilogue=epi, out=None if epi == 2 else out, w_up=w if epi == 2 else None))
+    assert [n for n in names if "gemm" in n]
+    assert any("gemm_wide" in n for n in names) == wide, names
