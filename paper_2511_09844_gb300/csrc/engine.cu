@@ -51,7 +51,7 @@ struct Model {
   }
 };
 
-constexpr int kLenClasses = 3;            // classes of prompt lengths, each with its own step graph
+constexpr int kLenClasses = 3;            // classes of context lengths, each with its own step graph
 
 struct Plan {
   int M = 0;
@@ -131,8 +131,8 @@ struct sd2_ctx {
   const int* logit_rows_d1 = nullptr;
   // graphs
   bool use_graphs = true;
-  cudaGraphExec_t g_step[kLenClasses] = {}, g_accept = nullptr;   // a step graph per class of prompt lengths
-  int len_class = 0;                      // of the last prefill (len_class_of)
+  cudaGraphExec_t g_step[kLenClasses] = {}, g_accept = nullptr;   // a step graph per class of context lengths
+  int longest = 0, steps = 0;             // the last prefill's longest prompt, and the steps since
   // profiling
   bool prof = false;
   bool stage_on = false;                  // stage markers inside the step (graph event nodes)
@@ -759,9 +759,14 @@ void drop_graphs(sd2_ctx* c) {
   c->g_accept = nullptr;
 }
 
-// Classes of the longest prompt, each with its own step graph: what the attention of a step runs on is
-// chosen by the context that it will see (AttnArgs::ctx), not by max_ctx alone, which is a capacity.
-int len_class_of(int maxlen) { return maxlen < 1024 ? 0 : maxlen < 4096 ? 1 : 2; }
+// Classes of the longest context, each with its own step graph (captured when a step first meets it): what the
+// attention of a step runs on is chosen by the context that it will see (AttnArgs::ctx), not by max_ctx alone, which
+// is a capacity. The lengths live on the device; a step commits 1 to k + 1 tokens a sequence, so the longest sequence
+// is taken to have grown by their mean a step. (sd2_generate could count, but is to run as the step loop does.)
+int len_class_of(int len) { return len < 1024 ? 0 : len < 4096 ? 1 : 2; }
+int expected_len(const sd2_ctx* c) {
+  return static_cast<int>(std::min<long>(c->cfg.max_ctx, c->longest + static_cast<long>(c->steps) * (c->cfg.k + 2) / 2));
+}
 int ctx_of_class(int len_class, int max_ctx) { return len_class == 2 ? max_ctx : std::min(max_ctx, len_class == 1 ? 1024 : 512); }
 
 // Context positions per attention split: whole 64-position tiles, at most attention_max_splits()
@@ -1041,8 +1046,8 @@ sd2_status sd2_prefill(sd2_ctx* c, int32_t batch, const int32_t* d_tokens, const
   c->p_v.pre_len = c->state;
   c->p_v.pre_stable = -1;
   c->p_v.pre_fresh = k + 1;
-  c->len_class = len_class_of(maxlen);
-  c->p_d1.ctx = c->p_dn.ctx = c->p_v.ctx = ctx_of_class(c->len_class, c->cfg.max_ctx);
+  c->longest = maxlen;
+  c->steps = 0;
   c->logit_rows_d1 = S + o_lr1;
 
   // verifier over the prompts: logits of each last row -> row b*(k+1) of the target buffer
@@ -1078,8 +1083,10 @@ sd2_status sd2_step(sd2_ctx* c) {
     CK(cudaStreamSynchronize(c->st));
   }
   sd2_status s;
+  const int len_class = len_class_of(expected_len(c));
+  c->p_d1.ctx = c->p_dn.ctx = c->p_v.ctx = ctx_of_class(len_class, c->cfg.max_ctx);
   if (c->use_graphs && !c->prof) {
-    cudaGraphExec_t& g = c->g_step[c->len_class];
+    cudaGraphExec_t& g = c->g_step[len_class];
     if (!g && (s = capture(c, &g, [&] { return run_step(c); })) != SD2_OK) return s;
     CK(cudaGraphLaunch(g, c->st));
   } else if ((s = run_step(c)) != SD2_OK) {
@@ -1087,6 +1094,7 @@ sd2_status sd2_step(sd2_ctx* c) {
   }
   if (c->stage_on) c->stage_done = true;
   if (c->gemm_timing) c->gemm_timing_done = true;
+  ++c->steps;
   c->phase = 2;
   return SD2_OK;
 }

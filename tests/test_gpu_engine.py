@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import parity
+from conftest import kernels_of
 from oracle import steering
 from oracle import model as omodel
 from paper_2511_09844_gb300 import sd2
@@ -345,3 +346,34 @@ def test_standalone_steering_of_any_batch(B):
     ref = torch.nn.functional.layer_norm(x, (dg,), st["ln_gamma"].double(), st["ln_beta"].double(), 1e-5)
     torch.testing.assert_close(out.double(), ref, atol=2e-5, rtol=2e-5)              # f32 sums of 192 and 128 terms
     torch.testing.assert_close(bias.double(), out.to(torch.bfloat16).double() @ st["w_s"].double().T, atol=2e-4, rtol=2e-5)
+
+
+def test_the_step_follows_the_context_as_it_grows():
+    """16 short prompts under a large max_ctx, 2 KV heads of 64: the drafter's attention starts on the kernel that
+    takes a short context whole and moves to split ones as the sequences pass 4096 positions."""
+    work = parity.tiny_work(k=16)
+    dev_w = [parity.to_device(w) for w in parity.tiny_weights(work)]
+    eng = sd2.SD2Engine(work, *dev_w, max_batch=16, max_ctx=8192, max_prefill_tokens=1024)
+    eng.prefill(W.make_prompts(work.verifier.vocab, 16, (20, 40), seed=50), [1.0] * 16, seed=51)
+
+    def iterate(n=1):
+        for _ in range(n):
+            eng.step()
+            eng.accept()
+
+    assert any("attn_few" in n for n in kernels_of(iterate))
+    iterate(4096 * 2 // 18)                 # a step commits 1 to 17 tokens: 9 on the mean
+    names = kernels_of(iterate)
+    assert names and not any("attn_few" in n for n in names), names
+    eng.check()
+    eng.close()
+
+
+@pytest.mark.parametrize("graphs", [True, False])
+def test_generation_across_a_length_class(graphs):
+    """A prompt that passes 1024 positions within a few steps: the steps before and after agree with the oracle."""
+    work = parity.tiny_work()
+    vw, dw, st = parity.tiny_weights(work)
+    prompts = W.make_prompts(work.verifier.vocab, 1, (1017, 1017), seed=52)
+    rep = parity.run(work, vw, dw, st, prompts, [1.0], seed=53, n_steps=6, max_ctx=4500, graphs=graphs)
+    assert rep.blocks == 6
