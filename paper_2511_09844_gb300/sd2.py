@@ -138,9 +138,15 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
+# The handle of a device's current stream without a Stream object around it (0.2 us a call, not 3.1): not a public
+# name of torch, so only used where torch has it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None):
-    # the handle of the current stream without a Stream object around it: 0.2 us a call, not 3.1
-    return stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if stream is None and _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())      # initialises CUDA, as current_stream() does
+    return (torch.cuda.current_stream() if stream is None else stream).cuda_stream
 
 
 def lm_config(shape) -> LMConfig:

@@ -151,3 +151,15 @@ def test_margin_of_the_approximate_normaliser_covers_its_error_terms(lib):
         rescales = (-(-V // 8192) + 1) * (ex2 + u)
         total = exponents + 4e-7 + sums + rescales
         assert total <= margin(V) < 2 * total + 1e-5, (V, total, margin(V))
+
+
+def test_the_current_stream_is_asked_for_as_torch_does(monkeypatch):
+    """The wrappers' default stream: CUDA is initialised first, so a child forked after that is refused with torch's
+    own message, and a torch without the raw handle is asked through the public name."""
+    import torch
+    monkeypatch.setattr(torch.cuda, "_is_in_bad_fork", lambda: True)
+    with pytest.raises(RuntimeError, match="forked subprocess"):
+        sd2._stream()
+    monkeypatch.setattr(sd2, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: type("S", (), {"cuda_stream": 7}))
+    assert sd2._stream() == 7 and sd2._stream(type("S", (), {"cuda_stream": 9})) == 9
