@@ -123,7 +123,9 @@ __global__ void __launch_bounds__(kThreads, BUF <= 3 ? 2 : 1) attn_few_kernel(co
   int pmax = -1;
 #pragma unroll
   for (int i = 0; i < kQv; ++i) pmax = max(pmax, sPos[i]);
-  if (tid == 0 && pmax + 1 > ctx_hi && a.err) atomicOr(a.err, static_cast<unsigned>(ERR_RANGE));
+  // A row beyond the planned bound or the block table is reported; what lies past the splits' cover is just not seen.
+  if (tid == 0 && min(static_cast<long>(pmax + 1), static_cast<long>(a.n_splits) * a.chunk) > ctx_hi && a.err)
+    atomicOr(a.err, static_cast<unsigned>(ERR_RANGE));
   const int hi = min(pmax + 1, w_hi), n = hi > w_lo ? (hi - w_lo + kSub - 1) / kSub : 0;
   const int pa = sPos[g8], pb = sPos[g8 + 8];          // this lane's two query vectors: g8 and g8 + 8
   uint32_t qa[kHd / 16][4];

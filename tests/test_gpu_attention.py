@@ -143,6 +143,28 @@ def test_row_beyond_the_planned_bound_is_reported():
     assert torch.isfinite(out).all()
 
 
+@pytest.mark.parametrize("hd,H,Hkv,n_seq,n_splits,chunk,kernel", [(64, 32, 8, 8, 4, 1024, "attn_few"), (128, 16, 4, 1, 16, 256, "attn_stream"),
+                                                                  (128, 16, 4, 1, 9, 128, "attn")])
+def test_rows_past_the_table_and_past_the_splits(hd, H, Hkv, n_seq, n_splits, chunk, kernel):
+    """Every kernel alike: a row at a position that the block table does not cover is reported; positions beyond
+    n_splits * chunk are not seen by a row that lies past them, and that is no error."""
+    L = 700 if n_splits != 16 else 4000
+    c = _case(14, [L] * n_seq, [1] * n_seq, H, Hkv, hd)
+    pre = dict(pre_len=[L - 1] * n_seq, pre_stable=0, pre_fresh=1)
+    assert _kernel(c, n_splits, chunk, **pre) == kernel
+    out, err = _run(c, n_splits, chunk, **pre)
+    assert err == 0
+    _check(out, _reference(c))
+    short = dict(c, table=c["table"][:, : L // 16 - 4].contiguous())
+    out, err = _run(short, n_splits, chunk, **pre)
+    assert err == ERR_RANGE and torch.isfinite(out).all()
+    fewer = 64 if n_splits == 9 else chunk * 3 // 4 if n_splits == 16 else 128       # n_splits * fewer < L
+    out, err = _run(c, n_splits, fewer, **pre)
+    assert err == 0
+    seen = dict(c, row_pos=torch.full_like(c["row_pos"], n_splits * fewer - 1))
+    _check(out, _reference(seen))
+
+
 def test_bad_arguments_are_rejected_on_the_host():
     c = _case(6, seq_lens=[100], rows_per_group=[2], H=32, Hkv=8, hd=128)
     with pytest.raises(sd2.SD2Error):
