@@ -117,8 +117,8 @@ def test_nonfinite_logits_are_reported_not_trapped():
     torch.cuda.synchronize()                      # no sticky error
 
 
-# More than 300 rows (B (2k + 1)) take the path that decides from approximate normalisers: rows whose
-# last group is partial, rows of 8-byte alignment (bf16, V % 8 == 4), vocabularies below one pass.
+# More than 152 rows (B (2k + 1); 96 of a vocabulary up to 65536) take the path that decides from approximate
+# normalisers, which all of these have: rows whose last group is partial, rows of 8-byte alignment (bf16, V % 8 == 4), vocabularies below one pass.
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("V,B,k", [(4, 110, 1), (36, 120, 3), (1004, 70, 4), (8196, 64, 2), (33000, 40, 4)])
 def test_many_rows_bit_exact(dtype, V, B, k):

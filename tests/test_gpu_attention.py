@@ -317,22 +317,33 @@ def test_prompt_scores_that_keep_rising():
                                          (64, 8, 2, 2), (64, 14, 2, 4), (64, 32, 8, 9), (64, 14, 2, 9)])
 @pytest.mark.parametrize("stable_off", [None, 0, 5])
 def test_long_context_kernel_beside_the_general_one(hd, H, Hkv, k1, stable_off):
-    """16 splits of 256 positions or more run on the long-context kernel, of 192 on the general one. 8 to 63
-    query vectors per KV head; contexts of one position, a block's and a tile's edge, one row past them, and
-    several tiles a split, with most splits empty at the short ones; with and without rows read early."""
+    """16 splits of 256 positions run on the long-context kernel, of 192 on the general one unless there are 48 or
+    more query vectors of 128 per KV head. 8 to 64 query vectors per KV head; contexts of one position, a block's
+    and a tile's edge, one row past them, and several tiles a split, with most splits empty at the short ones; with
+    and without rows read early. Two sequences a launch where there are 8 KV heads: more clusters of 16 than two
+    waves of them stay on the general kernel."""
     lens = [k1, 16 + k1, 128, 129, 1153, 2999]
-    c = _case(20, seq_lens=lens, rows_per_group=[k1] * len(lens), H=H, Hkv=Hkv, hd=hd)
-    ref = _reference(c)
-    kw = {}
-    if stable_off is not None:
-        kw = dict(pre_len=[max(0, L - k1 + 1 - stable_off) for L in lens], pre_stable=-1, pre_fresh=k1 + stable_off + 1)
-    outs = []
-    for n_splits, chunk in ((16, 192), (16, 256), (6, 1024), (1, 4096)):
-        out, err = _run(c, n_splits, chunk, **kw)
-        assert err == 0
-        _check(out, ref)
-        outs.append(out)
-    torch.testing.assert_close(outs[1], outs[0], atol=1.5e-2, rtol=1e-2)
+    N = k1 * (H // Hkv)
+    per = 2 if Hkv == 8 else 6
+    for i in range(0, 6, per):
+        some = lens[i:i + per]
+        c = _case(20 + i, seq_lens=some, rows_per_group=[k1] * per, H=H, Hkv=Hkv, hd=hd)
+        ref = _reference(c)
+        kw = {}
+        if stable_off is not None:
+            kw = dict(pre_len=[max(0, L - k1 + 1 - stable_off) for L in some], pre_stable=-1, pre_fresh=k1 + stable_off + 1)
+        wide = hd == 128 and N > 32
+        whole = "attn_prompt" if stable_off is None and N > 32 else "attn_stream"
+        outs = []
+        for n_splits, chunk, kernel in ((16, 192, "attn_stream" if wide else "attn"), (16, 256, "attn_stream"),
+                                        (6, 1024, "attn_stream"), (1, 4096, whole)):
+            if i == 0:
+                assert _kernel(c, n_splits, chunk, **kw) == kernel, (n_splits, chunk)
+            out, err = _run(c, n_splits, chunk, **kw)
+            assert err == 0
+            _check(out, ref)
+            outs.append(out)
+        torch.testing.assert_close(outs[1], outs[0], atol=1.5e-2, rtol=1e-2)
 
 
 @pytest.mark.parametrize("hd,k1,slots,spread", [(128, 1, 38, 12), (128, 4, 38, 12), (128, 9, 38, 12), (128, 16, 38, 12), (64, 9, 36, 24)])
@@ -343,6 +354,7 @@ def test_flat_mode_long_context_kernel(hd, k1, slots, spread):
     c = _case(21, seq_lens=lens, rows_per_group=[k1] * 13, H=8, Hkv=2, hd=hd)
     ref = _reference(c)
     ws = torch.zeros(sd2.load_library().sd2_attention_flat_workspace_bytes(2, slots, hd), dtype=torch.uint8, device="cuda")
+    assert _kernel(c, slots, 64 * spread + 64, [L - k1 + 1 for L in lens], -1, k1 + 1, run=_run_flat) == "attn_stream"
     for _ in range(2):
         out, err = _run_flat(c, slots, 64 * spread + 64, [L - k1 + 1 for L in lens], -1, k1 + 1, workspace=ws)
         assert err == 0
@@ -375,9 +387,9 @@ def test_prompt_rows_four_groups_a_cta(hd, H, Hkv, lens, first):
     _check(out, _prompt_reference(c))
 
 
-def _kernel(c, *args, **kw):
+def _kernel(c, *args, run=_run, **kw):
     """The attention kernel a launch of c runs on."""
-    names = [n for n in kernels_of(lambda: _run(c, *args, **kw)) if "attn" in n]
+    names = [n for n in kernels_of(lambda: run(c, *args, **kw)) if "attn" in n]
     assert len(names) == 1, names
     return next(k for k in ("attn_prompt", "attn_few", "attn_stream", "attn") if k + "_kernel" in names[0])
 
@@ -397,20 +409,23 @@ def test_short_prompts_run_on_the_general_kernel(hd, H, Hkv, lens, kernel):
 @pytest.mark.parametrize("stable_off", [0, 5])
 def test_few_query_vectors_over_many_sequences(H, Hkv, k1, n_seq, stable_off):
     """Heads of 64, 4 to 16 query vectors, 64 CTAs and more (one and two to an SM): the kernel for few query
-    vectors, beside the general one (which launches without pre-step lengths run on). Contexts of one row, of a
+    vectors, beside the general one (without pre-step lengths, in more clusters of 16 than two waves hold). Contexts of one row, of a
     cache block's edges, shorter than the warps, of a warp's 32 blocks and one more, ragged; then flat mode."""
     edges = [k1, 16, 17, 127 + k1, 129, 8 * 16 * 6, 8 * 16 * 6 + 1, 4097 + k1]
     lens = [max(k1, edges[i] if i < len(edges) else 20 + (131 * i) % 700) for i in range(n_seq)]
     c = _case(24, lens, [k1] * n_seq, H, Hkv, 64)
     ref = _reference(c)
     kw = dict(pre_len=[max(0, L - k1 + 1 - stable_off) for L in lens], pre_stable=-1, pre_fresh=k1 + stable_off + 1)
+    assert _kernel(c, 4, 1088, **kw) == "attn_few" and _kernel(c, 16, 320) == "attn"
     out, err = _run(c, 4, 1088, **kw)
     assert err == 0
     _check(out, ref)
-    other, err = _run(c, 4, 1088)
+    other, err = _run(c, 16, 320)
     assert err == 0
+    _check(other, ref)
     torch.testing.assert_close(out, other, atol=1.5e-2, rtol=1e-2)
     if n_seq * Hkv >= 128:
+        assert _kernel(c, n_seq, max(lens) + 16, kw["pre_len"], -1, kw["pre_fresh"], run=_run_flat) == "attn_few"
         out, err = _run_flat(c, n_seq, max(lens) + 16, kw["pre_len"], -1, kw["pre_fresh"])
         assert err == 0
         _check(out, ref)

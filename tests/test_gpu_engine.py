@@ -320,10 +320,10 @@ def test_standalone_steering_full_width(B):
 
 
 @pytest.mark.parametrize("heads,kv_heads,hd", [(4, 4, 64), (2, 2, 128), (6, 2, 64), (3, 1, 128)])
-@pytest.mark.parametrize("lens", [(43, 44), (342, 342), (260, 517)])
+@pytest.mark.parametrize("lens", [(43, 44), (65, 66), (342, 342), (260, 517)])
 def test_prompt_projections_on_cta_pairs(heads, kv_heads, hd, lens):
-    """Prompts of 129 rows, 1026 and about as many: q, k and v (2 to 3 weight tiles, the last one partial for 6 and 3
-    heads) through the CTA-pair GEMM, from 1024 rows on with the epilogue that rotates and appends to the paged
+    """Prompts of 129 rows, 195, 1026 and about as many: q, k and v (2 to 3 weight tiles, the last one partial for 6
+    and 3 heads) through the CTA-pair GEMM (their few features from 193 rows on), from 1024 rows on with the epilogue that rotates and appends to the paged
     cache; the decode steps that follow read it back."""
     base = parity.tiny_work()
     work = dataclasses.replace(base, verifier=W.shrink(base.verifier, n_heads=heads, n_kv_heads=kv_heads, head_dim=hd), batch=3)

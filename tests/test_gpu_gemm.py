@@ -160,7 +160,7 @@ def test_many_rows_of_half_a_feature_tile():
 
 
 @pytest.mark.parametrize("M,N,K", [(33, 512, 2048), (65, 4096, 1024), (72, 2048, 1536), (97, 3072, 1024), (127, 4096, 4096),
-                                   (128, 2560, 1280), (144, 4096, 2048), (141, 6144, 1024)])
+                                   (128, 2560, 1280), (144, 4096, 2048), (141, 4480, 1024), (141, 6144, 1024)])
 @pytest.mark.parametrize("with_bias", [False, True])
 def test_residual_add_of_several_owner_passes(M, N, K, with_bias):
     """Split-K tiles of 16 to 72 owned pairs and odd column counts: the owners' passes over four columns, one pass
