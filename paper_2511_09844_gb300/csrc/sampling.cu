@@ -254,15 +254,14 @@ __global__ void __launch_bounds__(kRowThreads) row_stats_kernel(const T* target,
       const int v = lo + (u * kRowThreads + static_cast<int>(threadIdx.x)) * 8;
       load8<T>(row, v, max(0, hi - v), z[u]);
     }
-  // Every CTA of the cluster runs: a store into the shared memory of one that has not started would be lost (a
-  // short vocabulary leaves slices empty, whose CTAs are at their stores at once). The row's loads are under way.
-  __syncwarp();
-  cluster_wait();
   if (rank == 0) prepare_race(r, B, k, sc, err, reset_err);
-  if (stopped && stopped[rr.b]) return;              // uniform over the cluster
   const float t = temp[rr.b];
   const bool greedy = !(t > 0.f);
-  if (greedy && rr.is_draft) return;
+  if ((stopped && stopped[rr.b]) || (greedy && rr.is_draft)) {   // uniform over the cluster
+    __syncwarp();
+    cluster_wait();
+    return;
+  }
   const float invT = greedy ? 1.f : inv_temp(t);
   bool bad;
   unsigned long long best;
@@ -288,6 +287,9 @@ __global__ void __launch_bounds__(kRowThreads) row_stats_kernel(const T* target,
   }
   best = block_max_u64(best, red);
   const int any_bad = __syncthreads_or(bad ? 1 : 0);
+  // Every CTA of the cluster runs: a store into the shared memory of one that has not started would be lost (a
+  // short vocabulary leaves slices empty, whose CTAs are here at once).
+  cluster_wait();
   if (threadIdx.x < C)
     st_dsmem_v4(static_cast<uint32_t>(__cvta_generic_to_shared(&sMax[rank])), threadIdx.x,
                 __uint_as_float(static_cast<uint32_t>(best)), __uint_as_float(static_cast<uint32_t>(best >> 32)),
