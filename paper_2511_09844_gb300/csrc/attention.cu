@@ -845,6 +845,11 @@ int attention_max_clusters(const AttnArgs& a) {
   return 0;
 }
 
+int attention_route(const AttnArgs& a) {
+  return attention_prompt_takes(a) ? ATTN_PROMPT : attention_few_takes(a) ? ATTN_FEW
+         : attention_stream_takes(a) ? ATTN_STREAM : ATTN_GENERAL;
+}
+
 cudaError_t attention(const AttnArgs& a, cudaStream_t st) {
   if (a.n_groups <= 0) return cudaSuccess;
   if (a.n_splits < 1 || a.n_splits > kMaxSplits || a.chunk <= 0 || a.chunk % kTile != 0) return cudaErrorInvalidValue;
@@ -855,9 +860,12 @@ cudaError_t attention(const AttnArgs& a, cudaStream_t st) {
                      a.chunk < 2 * kTile ||   // a ring of two tiles holds the merge's weights
                      !a.flat_acc || !a.flat_ml || !a.flat_cnt))
     return cudaErrorInvalidValue;
-  if (attention_prompt_takes(a)) return attention_prompt(a, st);
-  if (attention_few_takes(a)) return attention_few(a, st);
-  if (attention_stream_takes(a)) return attention_stream(a, st);
+  switch (attention_route(a)) {
+    case ATTN_PROMPT: return attention_prompt(a, st);
+    case ATTN_FEW: return attention_few(a, st);
+    case ATTN_STREAM: return attention_stream(a, st);
+    default: break;
+  }
   if (a.hd == 128) return launch<128>(a, st);
   if (a.hd == 64) return launch<64>(a, st);
   return cudaErrorInvalidValue;

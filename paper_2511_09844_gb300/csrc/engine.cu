@@ -14,6 +14,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <string>
 #include <vector>
@@ -51,7 +52,9 @@ struct Model {
   }
 };
 
-constexpr int kLenClasses = 3;            // classes of context lengths, each with its own step graph
+// What the attention launches of a step's three plans depend on beside the plans: kernel, splits, chunk, clusters
+// along the context, flat slots of each.
+using AttnRoutes = std::array<int, 15>;
 
 struct Plan {
   int M = 0;
@@ -131,7 +134,9 @@ struct sd2_ctx {
   const int* logit_rows_d1 = nullptr;
   // graphs
   bool use_graphs = true;
-  cudaGraphExec_t g_step[kLenClasses] = {}, g_accept = nullptr;   // a step graph per class of context lengths
+  std::vector<std::pair<AttnRoutes, cudaGraphExec_t>> g_steps;   // a step graph for each that was met
+  cudaGraphExec_t g_step = nullptr, g_accept = nullptr;          // g_step: of g_steps, the last step's
+  int len_class = -1;                     // the class of context lengths it was taken for
   int longest = 0, steps = 0;             // the last prefill's longest prompt, and the steps since
   // profiling
   bool prof = false;
@@ -383,6 +388,81 @@ sd2_status forward_chain(sd2_ctx* c, const Model& m, const Plan& p, const FwdOut
   return head(c, m, p, o);
 }
 
+// The attention launch of layer l of m over plan p.
+AttnArgs attn_args(sd2_ctx* c, const Model& m, const Plan& p, int l) {
+  const int M = p.M, H = m.c.n_heads, Hkv = m.c.n_kv_heads, hd = m.c.head_dim;
+  AttnArgs at{};
+  at.q = c->q; at.kv = m.cache(); at.layer = l; at.row_pos = p.pos;
+  at.grp_row0 = p.g_row0; at.grp_nrows = p.g_nrows; at.grp_seq = p.g_seq; at.n_groups = p.n_groups;
+  at.M = M; at.H = H; at.hd = hd; at.n_splits = p.n_splits; at.chunk = p.chunk; at.max_rows = p.max_rows; at.out = c->attn;
+  if (p.pre_len) {   // decode step: as many context splits as the GPU holds resident at once, no more
+    const long resident = static_cast<long>(attention_ctas_per_sm(hd)) * sm_count_cached();
+    const int want = std::max(1, static_cast<int>(resident / std::max(1, p.n_groups * Hkv)));
+    const int max_ctx = c->cfg.max_ctx;
+    auto chunk_for = [max_ctx](int ns, int R) { return 64 * ((max_ctx + 64 * ns * R - 1) / (64 * ns * R)); };
+    at.pre_len = p.pre_len;
+    at.ctx = p.ctx;
+    const int W = static_cast<int>(resident / Hkv);
+    if (p.n_groups >= kMinFlatGroups && p.n_groups <= kMaxFlatGroups && p.max_rows >= kMinFlatRows &&
+        W >= p.n_groups && max_ctx > 64) {
+      // many row groups (sequences of ragged lengths) of several rows each: flat mode, every
+      // resident CTA a slot, the slots shared out on the device by the sequences' lengths
+      at.n_splits = 1;
+      at.flat = W;
+      at.chunk = 64 * ((max_ctx + 63) / 64);
+      at.flat_acc = c->attn_flat_acc; at.flat_ml = c->attn_flat_ml; at.flat_cnt = c->attn_flat_cnt;
+    } else if (want < at.n_splits) {
+      at.n_splits = want;
+      at.chunk = chunk_for(want, 1);
+    } else if (at.n_splits < attention_max_splits()) {
+      // fewer planned splits than a cluster holds (the plan rounds its chunk up to whole tiles):
+      // a cluster's worth anyway; the kernel shares the step's actual context over them, so at
+      // short contexts a split holds one tile instead of two (batch 1 at context ~650: 6.78 -> 6.67 ms)
+      const int ns = std::min(attention_max_splits(), want);
+      at.n_splits = ns;
+      at.chunk = chunk_for(ns, 1);
+    } else if (at.n_splits >= 2 && p.n_groups <= kMaxCtxGroups && (hd != 128 || !attention_stream_takes(at))) {
+      // long contexts, unless the long-context kernel takes them: R clusters of 8 splits share the
+      // context, R as large as keeps every CTA at
+      // 4 or more tiles of 64 positions, the clusters within what the occupancy calculator says
+      // the device holds at once and the CTAs within 3/4 of the per-SM count. Measured on this kernel's
+      // 16K-context step, where the calculator allows 36 clusters of 8 at two CTAs per SM: the
+      // 8B verify's 32 clusters (256 CTAs, the per-SM count's 304 nearly full) still ran partly in
+      // a second wave, 24 did not (4.25 -> 3.84 ms); the 1B drafter's 32 (of 608) did not (step
+      // 1.02 -> 0.93 ms); clusters of 16 lost to clusters of 8 at every CTA count. One cluster of 16
+      // of the long-context kernel instead: heads of 128 (verify) 3.73 -> 3.49 ms, heads of 64 (five
+      // drafter steps) 4.56 -> 4.61 ms, so those stay.
+      const int ns = std::min(at.n_splits, 8);
+      int best_R = 0;
+      for (int Rc = 1; Rc <= kMaxCtxClusters; ++Rc) {
+        const long per_head = static_cast<long>(ns) * Rc;
+        if (4 * per_head * p.n_groups * Hkv > 3 * resident || max_ctx < 64 * 4 * per_head) break;
+        AttnArgs t = at;
+        t.n_splits = ns; t.n_ctx_clusters = Rc; t.chunk = chunk_for(ns, Rc);
+        t.part_acc = c->attn_part_acc; t.part_ml = c->attn_part_ml; t.part_cnt = c->attn_part_cnt;
+        // (not monotone in R: more CTAs per SM take less shared memory each)
+        if (static_cast<long>(Rc) * p.n_groups * Hkv > attention_max_clusters(t)) continue;
+        best_R = Rc;
+      }
+      if (best_R >= 2 && ns * best_R > at.n_splits) {   // else the planned single cluster
+        at.n_splits = ns;
+        at.n_ctx_clusters = best_R;
+        at.chunk = chunk_for(ns, best_R);
+        at.part_acc = c->attn_part_acc; at.part_ml = c->attn_part_ml; at.part_cnt = c->attn_part_cnt;
+      }
+    }
+    // a single cluster per (group, KV head) whose clusters cannot all be resident at once would
+    // run in two waves: fewer splits instead
+    while (at.n_ctx_clusters == 1 && at.n_splits > 1 &&
+           static_cast<long>(p.n_groups) * Hkv > attention_max_clusters(at)) {
+      --at.n_splits;
+      at.chunk = chunk_for(at.n_splits, 1);
+    }
+  }
+  at.pre_len = p.pre_len; at.pre_stable = p.pre_stable; at.pre_fresh = p.pre_fresh; at.err = c->errw;
+  return at;
+}
+
 // Decoder forward pass over the rows of plan p. On the tensor-core path the RMSNorm in front of
 // each projection is fused into the GEMMs around it: the residual-adding GEMM (or the embedding)
 // that produces x also writes bf16(x * gamma) and per-slice sums of squares of x, and the next
@@ -510,75 +590,7 @@ sd2_status forward(sd2_ctx* c, const Model& m, const Plan& p, const FwdOut& o) {
       }
     }
     if (fused) parts = gemm_norm_parts(go);
-    AttnArgs at{};
-    at.q = c->q; at.kv = m.cache(); at.layer = l; at.row_pos = p.pos;
-    at.grp_row0 = p.g_row0; at.grp_nrows = p.g_nrows; at.grp_seq = p.g_seq; at.n_groups = p.n_groups;
-    at.M = M; at.H = H; at.hd = hd; at.n_splits = p.n_splits; at.chunk = p.chunk; at.max_rows = p.max_rows; at.out = c->attn;
-    if (p.pre_len) {   // decode step: as many context splits as the GPU holds resident at once, no more
-      const long resident = static_cast<long>(attention_ctas_per_sm(hd)) * sm_count_cached();
-      const int want = std::max(1, static_cast<int>(resident / std::max(1, p.n_groups * Hkv)));
-      const int max_ctx = c->cfg.max_ctx;
-      auto chunk_for = [max_ctx](int ns, int R) { return 64 * ((max_ctx + 64 * ns * R - 1) / (64 * ns * R)); };
-      at.pre_len = p.pre_len;
-      at.ctx = p.ctx;
-      const int W = static_cast<int>(resident / Hkv);
-      if (p.n_groups >= kMinFlatGroups && p.n_groups <= kMaxFlatGroups && p.max_rows >= kMinFlatRows &&
-          W >= p.n_groups && max_ctx > 64) {
-        // many row groups (sequences of ragged lengths) of several rows each: flat mode, every
-        // resident CTA a slot, the slots shared out on the device by the sequences' lengths
-        at.n_splits = 1;
-        at.flat = W;
-        at.chunk = 64 * ((max_ctx + 63) / 64);
-        at.flat_acc = c->attn_flat_acc; at.flat_ml = c->attn_flat_ml; at.flat_cnt = c->attn_flat_cnt;
-      } else if (want < at.n_splits) {
-        at.n_splits = want;
-        at.chunk = chunk_for(want, 1);
-      } else if (at.n_splits < attention_max_splits()) {
-        // fewer planned splits than a cluster holds (the plan rounds its chunk up to whole tiles):
-        // a cluster's worth anyway; the kernel shares the step's actual context over them, so at
-        // short contexts a split holds one tile instead of two (batch 1 at context ~650: 6.78 -> 6.67 ms)
-        const int ns = std::min(attention_max_splits(), want);
-        at.n_splits = ns;
-        at.chunk = chunk_for(ns, 1);
-      } else if (at.n_splits >= 2 && p.n_groups <= kMaxCtxGroups && (hd != 128 || !attention_stream_takes(at))) {
-        // long contexts, unless the long-context kernel takes them: R clusters of 8 splits share the
-        // context, R as large as keeps every CTA at
-        // 4 or more tiles of 64 positions, the clusters within what the occupancy calculator says
-        // the device holds at once and the CTAs within 3/4 of the per-SM count. Measured on this kernel's
-        // 16K-context step, where the calculator allows 36 clusters of 8 at two CTAs per SM: the
-        // 8B verify's 32 clusters (256 CTAs, the per-SM count's 304 nearly full) still ran partly in
-        // a second wave, 24 did not (4.25 -> 3.84 ms); the 1B drafter's 32 (of 608) did not (step
-        // 1.02 -> 0.93 ms); clusters of 16 lost to clusters of 8 at every CTA count. One cluster of 16
-        // of the long-context kernel instead: heads of 128 (verify) 3.73 -> 3.49 ms, heads of 64 (five
-        // drafter steps) 4.56 -> 4.61 ms, so those stay.
-        const int ns = std::min(at.n_splits, 8);
-        int best_R = 0;
-        for (int Rc = 1; Rc <= kMaxCtxClusters; ++Rc) {
-          const long per_head = static_cast<long>(ns) * Rc;
-          if (4 * per_head * p.n_groups * Hkv > 3 * resident || max_ctx < 64 * 4 * per_head) break;
-          AttnArgs t = at;
-          t.n_splits = ns; t.n_ctx_clusters = Rc; t.chunk = chunk_for(ns, Rc);
-          t.part_acc = c->attn_part_acc; t.part_ml = c->attn_part_ml; t.part_cnt = c->attn_part_cnt;
-          // (not monotone in R: more CTAs per SM take less shared memory each)
-          if (static_cast<long>(Rc) * p.n_groups * Hkv > attention_max_clusters(t)) continue;
-          best_R = Rc;
-        }
-        if (best_R >= 2 && ns * best_R > at.n_splits) {   // else the planned single cluster
-          at.n_splits = ns;
-          at.n_ctx_clusters = best_R;
-          at.chunk = chunk_for(ns, best_R);
-          at.part_acc = c->attn_part_acc; at.part_ml = c->attn_part_ml; at.part_cnt = c->attn_part_cnt;
-        }
-      }
-      // a single cluster per (group, KV head) whose clusters cannot all be resident at once would
-      // run in two waves: fewer splits instead
-      while (at.n_ctx_clusters == 1 && at.n_splits > 1 &&
-             static_cast<long>(p.n_groups) * Hkv > attention_max_clusters(at)) {
-        --at.n_splits;
-        at.chunk = chunk_for(at.n_splits, 1);
-      }
-    }
-    at.pre_len = p.pre_len; at.pre_stable = p.pre_stable; at.pre_fresh = p.pre_fresh; at.err = c->errw;
+    const AttnArgs at = attn_args(c, m, p, l);
     double kvb = 0;
     if (c->prof && !c->h_n.empty()) {
       for (int b = 0; b < c->B; ++b) kvb += 2.0 * 2.0 * Hkv * hd * (c->h_n[b] + 16);
@@ -751,23 +763,35 @@ sd2_status capture(sd2_ctx* c, cudaGraphExec_t* exec, F body) {
 }
 
 void drop_graphs(sd2_ctx* c) {
-  for (cudaGraphExec_t& g : c->g_step) {
-    if (g) cudaGraphExecDestroy(g);
-    g = nullptr;
-  }
+  for (auto& g : c->g_steps) cudaGraphExecDestroy(g.second);
+  c->g_steps.clear();
+  c->g_step = nullptr;
+  c->len_class = -1;
   if (c->g_accept) cudaGraphExecDestroy(c->g_accept);
   c->g_accept = nullptr;
 }
 
-// Classes of the longest context, each with its own step graph (captured when a step first meets it): what the
-// attention of a step runs on is chosen by the context that it will see (AttnArgs::ctx), not by max_ctx alone, which
-// is a capacity. The lengths live on the device; a step commits 1 to k + 1 tokens a sequence, so the longest sequence
-// is taken to have grown by their mean a step. (sd2_generate could count, but is to run as the step loop does.)
+// Classes of the longest context: what the attention of a step runs on is chosen by the context that it will see
+// (AttnArgs::ctx), not by max_ctx alone, which is a capacity. The lengths live on the device; a step commits 1 to
+// k + 1 tokens a sequence, so the longest sequence is taken to have grown by their mean a step. (sd2_generate could
+// count, but is to run as the step loop does.) A step graph is captured when a class first asks for other launches
+// than those captured (8B/1B: a capture takes 2 ms at batch 1, 4 at 16).
 int len_class_of(int len) { return len < 1024 ? 0 : len < 4096 ? 1 : 2; }
 int expected_len(const sd2_ctx* c) {
   return static_cast<int>(std::min<long>(c->cfg.max_ctx, c->longest + static_cast<long>(c->steps) * (c->cfg.k + 2) / 2));
 }
 int ctx_of_class(int len_class, int max_ctx) { return len_class == 2 ? max_ctx : std::min(max_ctx, len_class == 1 ? 1024 : 512); }
+
+AttnRoutes step_routes(sd2_ctx* c) {
+  AttnRoutes r{};
+  int i = 0;
+  for (const Plan* p : {&c->p_d1, &c->p_dn, &c->p_v}) {
+    const Model& m = p == &c->p_v ? c->V : c->D;
+    const AttnArgs a = attn_args(c, m, *p, m.c.n_layers - 1);
+    for (int v : {attention_route(a), a.n_splits, a.chunk, a.n_ctx_clusters, a.flat}) r[i++] = v;
+  }
+  return r;
+}
 
 // Context positions per attention split: whole 64-position tiles, at most attention_max_splits()
 // splits (one cluster).
@@ -1086,9 +1110,19 @@ sd2_status sd2_step(sd2_ctx* c) {
   const int len_class = len_class_of(expected_len(c));
   c->p_d1.ctx = c->p_dn.ctx = c->p_v.ctx = ctx_of_class(len_class, c->cfg.max_ctx);
   if (c->use_graphs && !c->prof) {
-    cudaGraphExec_t& g = c->g_step[len_class];
-    if (!g && (s = capture(c, &g, [&] { return run_step(c); })) != SD2_OK) return s;
-    CK(cudaGraphLaunch(g, c->st));
+    if (len_class != c->len_class) {
+      const AttnRoutes routes = step_routes(c);
+      cudaGraphExec_t g = nullptr;
+      for (const auto& have : c->g_steps)
+        if (have.first == routes) g = have.second;
+      if (!g) {
+        if ((s = capture(c, &g, [&] { return run_step(c); })) != SD2_OK) return s;
+        c->g_steps.push_back({routes, g});
+      }
+      c->g_step = g;
+      c->len_class = len_class;
+    }
+    CK(cudaGraphLaunch(c->g_step, c->st));
   } else if ((s = run_step(c)) != SD2_OK) {
     return s;
   }

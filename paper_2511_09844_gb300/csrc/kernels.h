@@ -150,8 +150,8 @@ cudaError_t gemm_wide(const GemmArgs& g, unsigned* err, cudaStream_t st);
 // once per (pointer, shape), and an activation [rows, K] with row stride ld.
 bool gemm_weight_map(void* map, const void* w, int rows, int K, int box_rows);
 bool gemm_row_map(void* map, const void* x, int rows, int K, int ld, int box_rows);
-// Clusters of `size` CTAs of 192 threads (a GEMM's, or the long-context attention's) with `smem` bytes
-// of dynamic shared memory that are resident at once.
+// Clusters of `size` CTAs with `smem` bytes of dynamic shared memory that are resident at once, for kernels that
+// shared memory bounds: the GEMMs' (192 and 320 threads) and the long-context attention's (256).
 int gemm_max_clusters(int size, int smem);
 
 // 2-D bf16 TMA map (CUtensorMap, 128 bytes) of a row-major [rows, K] weight: boxes of box_rows x 64
@@ -242,6 +242,9 @@ struct AttnArgs {
   int ctx = 0;
 };
 cudaError_t attention(const AttnArgs& a, cudaStream_t st);
+// The kernel that attention() runs these (valid) arguments on.
+enum { ATTN_GENERAL, ATTN_PROMPT, ATTN_FEW, ATTN_STREAM };
+int attention_route(const AttnArgs& a);
 // The tcgen05 kernel for prompt rows (attn_prompt.cu); attention() runs it for the launches that
 // attention_prompt_takes accepts.
 bool attention_prompt_takes(const AttnArgs& a);
