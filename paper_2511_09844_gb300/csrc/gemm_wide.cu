@@ -14,8 +14,9 @@
 // It takes over from the weights-as-M kernel of gemm_tc.cu above 128 rows (kWideMinRows): there a
 // 128-row gate/up of the 8B width is still as fast (53.0 against 52.4 us), 144 rows are not (64.1
 // against 51.7), and its whole-tile epilogue, 16 columns at a time with dependent loads and stores,
-// made 256 rows x 14336 -> 4096 231 us (34.9 here). Gate/up of 2000 rows x 4096 -> 2 x 14336:
-// 394 -> 252 us (1.86 PFLOP/s; cuBLAS reaches 1.98 on 8192^3), 8000 rows 1507 -> 989; 8000 rows
+// made 256 rows x 14336 -> 4096 231 us (34.9 here). Gate/up of 2000 rows x 4096 -> 2 x 14336: in a
+// short burst 394 -> 252 us (1.86 PFLOP/s; cuBLAS 1.94 on 8192^3), in a long run, at the clocks that
+// the power limit leaves, 420 -> 290 (1.62; cuBLAS 1.75); bursts of 8000 rows 1507 -> 989; 8000 rows
 // x 14336 -> 4096 1009 -> 522; x 4096 -> 6144 280 -> 235. Prefill of 8352 prompt tokens through the
 // 8B/1B pair 206 -> 100 ms, of 512 25.6 -> 9.7.
 // Between 129 and 192 rows short and very long weight matrices stay there (weights_as_m_rows).
@@ -188,13 +189,9 @@ __device__ __forceinline__ unsigned long long wide_ns() {
   return t;
 }
 __device__ __forceinline__ float silu(float y) { return y / (1.f + __expf(-y)); }
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
 // 8 f32 as 8 bf16
 __device__ __forceinline__ uint4 pack8(const float* v) {
-  return make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+  return make_uint4(bf16_pair(v[0], v[1]), bf16_pair(v[2], v[3]), bf16_pair(v[4], v[5]), bf16_pair(v[6], v[7]));
 }
 
 // Tile t -> (token tile, weight tile): groups of kGroupTiles token tiles, weight tiles slowest.
@@ -253,7 +250,7 @@ __device__ __forceinline__ void emit_rows(const WideArgs& a, float4* patch, int 
     if (E == EPI_ADD && a.norm_out) {
       ss[i] += (y.x * y.x + y.y * y.y) + (y.z * y.z + y.w * y.w);
       *reinterpret_cast<uint2*>(a.norm_out + at) =
-          make_uint2(pack2(y.x * bf_lo(o.g.x), y.y * bf_hi(o.g.x)), pack2(y.z * bf_lo(o.g.y), y.w * bf_hi(o.g.y)));
+          make_uint2(bf16_pair(y.x * bf_lo(o.g.x), y.y * bf_hi(o.g.x)), bf16_pair(y.z * bf_lo(o.g.y), y.w * bf_hi(o.g.y)));
       if (a.tap_mask) {
         const int tr = a.tap_row ? a.tap_row[m] : m;
         if (tr >= 0)
