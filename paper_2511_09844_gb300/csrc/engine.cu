@@ -430,8 +430,8 @@ AttnArgs attn_args(sd2_ctx* c, const Model& m, const Plan& p, int l) {
       // 8B verify's 32 clusters (256 CTAs, the per-SM count's 304 nearly full) still ran partly in
       // a second wave, 24 did not (4.25 -> 3.84 ms); the 1B drafter's 32 (of 608) did not (step
       // 1.02 -> 0.93 ms); clusters of 16 lost to clusters of 8 at every CTA count. One cluster of 16
-      // of the long-context kernel instead: heads of 128 (verify) 3.73 -> 3.49 ms, heads of 64 (five
-      // drafter steps) 4.56 -> 4.61 ms, so those stay.
+      // of the long-context kernel instead: heads of 128 (verify) 3.73 -> 3.53 ms, heads of 64 (five
+      // drafter steps) 4.56 -> 4.61 ms and more since, so those stay.
       const int ns = std::min(at.n_splits, 8);
       int best_R = 0;
       for (int Rc = 1; Rc <= kMaxCtxClusters; ++Rc) {
