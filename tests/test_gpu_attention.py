@@ -455,3 +455,15 @@ def test_probabilities_enter_the_products_unrounded(kind, hd, H, Hkv, k1):
     assert err == 0
     rounding = (ref.to(torch.bfloat16).double() - ref).norm()
     assert (out.double() - ref).norm() <= 1.05 * rounding
+
+
+@pytest.mark.parametrize("hd,H,Hkv", [(128, 8, 2), (64, 14, 2)])
+@pytest.mark.parametrize("at", [0, 31, 32, 63, 64, 127, 128, 200, 511])
+def test_prompt_scores_that_jump(hd, H, Hkv, at):
+    """One key far above the others (its scores pass the reference by up to 2^80 either way), in every 32 positions
+    of a tile and in later tiles: what was formed of the tile before it is rescaled with the sums and O."""
+    c = _prompt_case(29, [512], [0], H, Hkv, hd)
+    c["pool"][:, int(c["table"][0, at // 16]), 0, :, at % 16] *= 12.0
+    out, err = _run(c, 1, 512, max_rows=64 // (H // Hkv))
+    assert err == 0
+    _check(out, _prompt_reference(c))
